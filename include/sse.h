@@ -323,15 +323,14 @@ int sse_barotropic_substep_noalloc(const sse_mesh *mesh, int order, double dt, i
 
 /* Launch-shape choices of a state.  patch_cells: target cells per patch of
  * the tiled barotropic sub-cycle.  0 (the default): one patch per SM, at most
- * one patch per 64 cells (an FP64 mesh of at most 512 cells: per 256).  A positive value asks for about that many cells per
+ * one patch per 64 cells.  A positive value asks for about that many cells per
  * patch, up to two patches per SM (more than one patch per SM run as 512-thread
  * blocks holding at most half an SM's shared memory each).  Larger patches use
  * fewer SMs for longer, which lets the sub-cycles of several states run side
  * by side.  bcl_patch_cells: cells per patch of the fused baroclinic kernel
  * (Algorithm 1), one of 160, 128, 112, 96, 80, 64, 48, 32; 0 (the default):
  * for a state stepped alone the largest patches that fill whole waves of the
- * GPU (an FP64 mesh of at most 512 cells: 112 cells), for states packed into
- * one launch the largest that fit the kernel with as many CTAs per SM as it is
+ * GPU, for states packed into one launch the largest that fit the kernel with as many CTAs per SM as it is
  * compiled for.  A size whose plan does not fit falls back to the default.
  * Smaller patches give a small mesh more CTAs (shorter latency when it runs
  * alone) at the cost of more halo work.  Results are the same bits for every
