@@ -319,8 +319,8 @@ constexpr int TILE_NE2 = 10;  // edgesOnEdge terms evaluated per edge (padding -
 //            the coefficients stream from L2
 // Per step on the level-7 sphere (three sub-cycles of 40 sub-steps): FP64, from
 // the global-memory kernel, 13.0 -> 7.2 ms, now bound by the FP64 pipe; FP32 1.68
-// -> 1.39 ms with the exchange and the term order, bound by its gathers, issue
-// and the barriers between its six phases.
+// -> 1.44 ms with the exchange written by the last stage, bound by its gathers,
+// issue and the barriers between its six phases.
 template <class R> struct TileSmem {
     R *u0, *ua, *uh, *fl, *z0, *za, *zh, *F0, *ub0, *d0, *d0h, *fz;
     unsigned int *c12;                // packed byte offsets of (c1, c2) into the cell arrays

@@ -78,84 +78,6 @@ void bisect(const std::vector<std::vector<int>> &adj, std::vector<int> cells, in
     bisect(adj, right, parts - p1, owner, next, mask, tagctr, da, db);
 }
 
-// Term order of one warp's gathers.  Entry i of the warp (n <= 32 entries) sums
-// nt[i] <= D terms; term t of entry i is a 4-byte word in shared-memory bank
-// bank[i * D + t].  An entry's terms may be summed in any order, so slot j of the
-// warp (its j-th gather) can take one term of every entry such that few banks
-// are asked for two words at once: slot[i * D + j] is the term that entry i
-// takes in slot j.  Starting from the given order, entries swap two of their
-// slots where that lowers the excess over the slots' allowed loads; a slot
-// allows one word per bank, or two where the fullest bank (which must be read as
-// often as its load) needs them.  Level-7 sphere, 152 patches: an edge's ten
-// gathers take 19.2 wavefronts instead of 23.5, a cell's six 11.0 instead of
-// 18.2 (the sub-cycle 1.44 -> 1.38 ms per step, mixed), for half a second more
-// on the host when the mesh's first state is made.
-void spread_terms(int n, int D, const int16_t *nt, const std::vector<int> &bank,
-                  std::vector<int> &slot) {
-    constexpr int B = 32;
-    int load[B] = {0}, most = 0;
-    for (int i = 0; i < n; i++)
-        for (int j = 0; j < nt[i]; j++) most = std::max(most, ++load[bank[i * D + j]]);
-    std::vector<int> first(n * D), cnt(D * B), best;
-    for (int x = 0; x < n * D; x++) first[x] = x % D;
-    auto count = [&](const std::vector<int> &s) {
-        std::fill(cnt.begin(), cnt.end(), 0);
-        for (int i = 0; i < n; i++)
-            for (int j = 0; j < nt[i]; j++) cnt[j * B + bank[i * D + s[i * D + j]]]++;
-    };
-    // wavefronts of the warp's gathers: each slot's fullest bank
-    auto waves = [&]() {
-        int t = 0;
-        for (int j = 0; j < D; j++) t += *std::max_element(&cnt[j * B], &cnt[j * B] + B);
-        return t;
-    };
-    count(first);
-    best = first;
-    int least = waves();
-    for (int T = std::max(D, most); T <= 2 * D && T < least; T += 2) {
-        std::vector<int> s = first;
-        auto excess = [&](int j, int c) {
-            const int o = c - (1 + (j < T - D ? 1 : 0));
-            return o > 0 ? o * o : 0;
-        };
-        count(s);
-        bool over = true;
-        for (int round = 0; round < 4 && over; round++) {
-            bool moved = false;
-            over = false;
-            for (int i = 0; i < n; i++)
-                for (int j = 0; j < nt[i]; j++) {
-                    const int bj = bank[i * D + s[i * D + j]];
-                    if (!excess(j, cnt[j * B + bj])) continue;
-                    over = true;
-                    int at = -1, gain = -1;
-                    for (int k = 0; k < nt[i]; k++) {
-                        const int bk = bank[i * D + s[i * D + k]];
-                        if (k == j || bk == bj) continue;
-                        const int a = cnt[j * B + bj], b = cnt[k * B + bk];
-                        const int c = cnt[k * B + bj], d = cnt[j * B + bk];
-                        const int g = excess(j, a) - excess(j, a - 1) + excess(k, b) - excess(k, b - 1) -
-                                      (excess(k, c + 1) - excess(k, c)) -
-                                      (excess(j, d + 1) - excess(j, d));
-                        if (g > gain) { gain = g; at = k; }
-                    }
-                    if (at < 0) continue;
-                    const int bk = bank[i * D + s[i * D + at]];
-                    cnt[j * B + bj]--; cnt[at * B + bk]--;
-                    cnt[at * B + bj]++; cnt[j * B + bk]++;
-                    std::swap(s[i * D + j], s[i * D + at]);
-                    moved = moved || gain > 0;
-                }
-            if (!moved && round > 2) break;
-        }
-        count(s);
-        const int t = waves();
-        if (t < least) { least = t; best = s; }
-        if (!over) break;
-    }
-    slot = best;
-}
-
 }  // namespace
 
 std::vector<int> partition_cells(const HostMesh &hm, int P) {
@@ -170,30 +92,6 @@ std::vector<int> partition_cells(const HostMesh &hm, int P) {
     int next = 0, tagctr = 0;
     bisect(adj, all, P, owner, next, mask, tagctr, da, db);
     return owner;
-}
-
-// The sub-cycle kernel's warps take 32 consecutive entries of a patch: the
-// terms of each warp's edges and cells in the order spread_terms finds.
-static void spread_patch_terms(const HostMesh &hm, TilePatch &tp) {
-    std::vector<int> bank, slot;
-    auto spread = [&](int count, int D, const std::vector<int16_t> &nt, std::vector<int16_t> &idx,
-                      std::vector<double> &coef) {
-        for (int w = 0; w < count; w += 32) {
-            const int m = std::min(32, count - w);
-            const size_t x0 = (size_t)w * D;
-            bank.resize((size_t)m * D);
-            for (int x = 0; x < m * D; x++) bank[x] = idx[x0 + x] % 32;
-            spread_terms(m, D, &nt[w], bank, slot);
-            const std::vector<int16_t> a(idx.begin() + x0, idx.begin() + x0 + m * D);
-            const std::vector<double> c(coef.begin() + x0, coef.begin() + x0 + m * D);
-            for (int x = 0; x < m * D; x++) {
-                idx[x0 + x] = a[x / D * D + slot[x]];
-                coef[x0 + x] = c[x / D * D + slot[x]];
-            }
-        }
-    };
-    spread(tp.ne, hm.maxE2, tp.n2, tp.eoe, tp.cfc);
-    spread(tp.nc, hm.maxE, tp.nce, tp.ce, tp.divc);
 }
 
 bool tile_stencil_ok(const HostMesh &hm) {
@@ -302,6 +200,13 @@ bool build_tile_plan(const HostMesh &hm, int P, int K, TilePlan &plan) {
             tp.c12[k] = (int32_t)((uint32_t)a | ((uint32_t)b << 16));
             tp.n2[k] = (int16_t)hm.neoe[e];
             tp.invdc[k] = hm.invdc[e];
+            // The terms of a sum keep the mesh's order in every patch that holds
+            // a copy of the edge (and of the cell, below), so that all copies
+            // round alike and no result depends on the patches.  (An order per
+            // patch that spreads a warp's gathers over the shared-memory banks
+            // takes 4% off the sub-cycle, level 7, but gives a halo copy other
+            // bits than its owner; one order per mesh chosen for the default
+            // patches keeps half of that there and loses on any others.)
             for (int j = 0; j < hm.neoe[e]; j++) {
                 const int ep = hm.eoe[(size_t)e * hm.maxE2 + j];
                 tp.eoe[(size_t)k * hm.maxE2 + j] = (int16_t)(le[ep] >= 0 ? le[ep] : dummyE);
@@ -323,7 +228,6 @@ bool build_tile_plan(const HostMesh &hm, int P, int K, TilePlan &plan) {
             }
         }
         tp.H[nc] = 1.0;  // dummy cell: finite depth
-        spread_patch_terms(hm, tp);
         // prefix counts by ring (owned edges have ring 0 or 1)
         for (int r = 0; r < 3; r++) {
             int n = tp.n_own_e;
