@@ -383,12 +383,12 @@ int sse_state_graphs(const sse_state *state, int *graphs);
 #define SSE_INJECT_BARRIER_STALL 1
 int sse_state_inject(sse_state *state, int what, int value);
 /* Autotuner: times the Algorithm 3/4 sub-cycle (M = 20) of a zero state of
- * this mesh for each candidate patch size, then Algorithm 1 for each fused
- * baroclinic patch size whose plan fits, and returns the best of each for the
- * objective (SSE_TUNE_*: LATENCY the fastest; THROUGHPUT the least SM-time,
- * duration x the SMs the launch holds, among candidates within twice the
- * fastest).  Runs GPU work on a private stream; the result is cached in the
- * mesh. */
+ * this mesh for the default and each candidate patch size, then Algorithm 1
+ * for the default and each fused baroclinic patch size whose plan fits, and
+ * returns the best of each for the objective (SSE_TUNE_*: LATENCY the fastest;
+ * THROUGHPUT the least SM-time, duration x the SMs the launch holds, among
+ * candidates within twice the fastest); 0 where that is the default.  Runs
+ * GPU work on a private stream; the result is cached in the mesh. */
 int sse_tune(const sse_mesh *mesh, const sse_params *params, int objective, sse_tuning *out);
 
 /* Device bytes a state of this mesh and parameter set would allocate
