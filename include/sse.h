@@ -393,12 +393,17 @@ int sse_tune(const sse_mesh *mesh, const sse_params *params, int objective, sse_
 
 /* Device bytes a state of this mesh and parameter set would allocate
  * (nothing is allocated here).  The read-only patch plans of the tiled and
- * fused kernels are not among them: the mesh holds one device copy per plan
- * and precision for all its states, made with the first state that needs it
- * and freed with the mesh. */
+ * fused kernels are not among them: the states of a mesh share one device copy
+ * per plan and precision (sse_mesh_plan_bytes). */
 int sse_state_footprint(const sse_mesh *mesh, const sse_params *params, size_t *bytes);
 int sse_state_footprint_ex(const sse_mesh *mesh, const sse_params *params,
                            const sse_tuning *tuning, size_t *bytes);
+
+/* Device bytes of the mesh's patch plans: one copy per plan and precision, made
+ * with the first state that needs it and kept for the states that follow.
+ * Copies that no state holds are freed with the mesh, behind sse_tune, and where
+ * device memory runs out while a state is made. */
+int sse_mesh_plan_bytes(const sse_mesh *mesh, size_t *bytes);
 
 /* dims = {nCells, nEdges, nVertices, nLayers} of a mesh. */
 int sse_mesh_dims(const sse_mesh *mesh, int32_t dims[4]);

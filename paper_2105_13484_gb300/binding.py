@@ -91,7 +91,7 @@ EXPORTS = ["sse_mesh_create", "sse_mesh_destroy", "sse_state_create", "sse_state
            "sse_state_inject",
            "sse_state_set_f32", "sse_state_get_f32", "sse_state_graphs", "sse_state_transfer",
            "sse_state_sync",
-           "sse_tune",
+           "sse_tune", "sse_mesh_plan_bytes",
            "sse_mesh_dims", "sse_server_create", "sse_server_submit", "sse_server_query",
            "sse_server_wait", "sse_server_stats", "sse_server_release", "sse_server_destroy",
            "sse_strerror"]
@@ -153,6 +153,7 @@ def load(path: str = LIB_PATH):
     lib.sse_state_inject.argtypes = [ct.c_void_p, ct.c_int, ct.c_int]
     lib.sse_state_set_f32.argtypes = [ct.c_void_p, ct.c_int, ct.c_void_p]
     lib.sse_state_get_f32.argtypes = [ct.c_void_p, ct.c_int, ct.c_void_p]
+    lib.sse_mesh_plan_bytes.argtypes = [ct.c_void_p, ct.POINTER(ct.c_size_t)]
     lib.sse_tune.argtypes = [ct.c_void_p, ct.POINTER(Params), ct.c_int, ct.POINTER(Tuning)]
     lib.sse_server_submit.argtypes = [ct.c_void_p, ct.c_void_p, ct.POINTER(Params), ct.c_void_p,
                                       ct.c_void_p, ct.c_void_p, ct.c_void_p, ct.c_int,
@@ -463,6 +464,13 @@ def footprint(mesh: Mesh, params: dict, precision="fp64", patch_cells: int = 0,
     _check(lib.sse_state_footprint_ex(mesh.handle, ct.byref(prm), ct.byref(t), ct.byref(out)),
            "sse_state_footprint_ex")
     return int(out.value)
+
+
+def plan_bytes(mesh: Mesh) -> int:
+    """Device bytes of the mesh's patch plans (sse_mesh_plan_bytes)."""
+    out = ct.c_size_t()
+    _check(load().sse_mesh_plan_bytes(mesh.handle, ct.byref(out)), "sse_mesh_plan_bytes")
+    return out.value
 
 
 def tune_shapes(mesh: Mesh, params: dict, precision="mixed", objective="throughput") -> dict:
