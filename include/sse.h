@@ -391,18 +391,20 @@ int sse_state_inject(sse_state *state, int what, int value);
  * GPU work on a private stream; the result is cached in the mesh. */
 int sse_tune(const sse_mesh *mesh, const sse_params *params, int objective, sse_tuning *out);
 
-/* Device bytes a state of this mesh and parameter set would allocate
- * (nothing is allocated here).  The read-only patch plans of the tiled and
- * fused kernels are not among them: the states of a mesh share one device copy
- * per plan and precision (sse_mesh_plan_bytes). */
+/* Device bytes a state of this mesh and parameter set may allocate (nothing is
+ * allocated here): its own arrays and the patch plans of the tiled and fused
+ * kernels, those of packed launches among them.  The states of a mesh share one
+ * device copy per plan and precision (sse_mesh_plan_bytes), so that several
+ * take less than the sum of their footprints. */
 int sse_state_footprint(const sse_mesh *mesh, const sse_params *params, size_t *bytes);
 int sse_state_footprint_ex(const sse_mesh *mesh, const sse_params *params,
                            const sse_tuning *tuning, size_t *bytes);
 
 /* Device bytes of the mesh's patch plans: one copy per plan and precision, made
  * with the first state that needs it and kept for the states that follow.
- * Copies that no state holds are freed with the mesh, behind sse_tune, and where
- * device memory runs out while a state is made. */
+ * Copies that no state holds are freed with the mesh, behind sse_tune, where
+ * device memory runs out while a state is made, and where they stand in the way
+ * of a request runtime's budget. */
 int sse_mesh_plan_bytes(const sse_mesh *mesh, size_t *bytes);
 
 /* dims = {nCells, nEdges, nVertices, nLayers} of a mesh. */
@@ -417,8 +419,9 @@ int sse_mesh_dims(const sse_mesh *mesh, int32_t dims[4]);
  * SSE_FIELD_WIND) advanced n_steps SSPRK{order}-SE steps
  * of dt with n_substeps barotropic sub-steps (Sec. 3.2 / 3.3).  A worker
  * thread admits requests in arrival order while the sum of their
- * sse_state_footprint stays within hbm_budget_bytes and at most max_active
- * run; each admitted request gets its own stream and a device-resident state
+ * sse_state_footprint (and of the plans that finished requests left on their
+ * meshes, which are freed first) stays within hbm_budget_bytes and at most
+ * max_active run; each admitted request gets its own stream and a device-resident state
  * and is advanced steps_per_launch steps at a time, its work overlapping with
  * that of the other active requests.  When it reaches its horizon the final
  * (u, h, tracers) are written to the caller's output buffers (same layouts;

@@ -5,8 +5,9 @@
 // follow, and kept when the last one goes, so that a state made later on the
 // mesh finds it (on the level-7 sphere a copy costs 42 ms to make, mixed, and
 // a state 8 without).  The idle copies are given back by trim(), which the
-// autotuner calls behind its candidates and state creation where memory has run
-// out, and with the store.  Nothing here synchronises the device: a copy is
+// autotuner calls behind its candidates, the request runtime where they stand in
+// the way of its budget and state creation where memory has run out, and with
+// the store.  Nothing here synchronises the device: a copy is
 // complete before any second state can see it, and is freed in stream order
 // behind the work of every state that held it.
 #pragma once

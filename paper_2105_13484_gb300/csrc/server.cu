@@ -2,8 +2,10 @@
 //
 // Requests (a mesh, parameters, an initial state, a scheme and a horizon of
 // n_steps large steps) are queued in arrival order.  One worker thread admits
-// them while their device footprint (sse_state_footprint) fits the HBM budget
-// and the active-slot limit, gives each admitted request its own non-blocking
+// them while their device footprint (sse_state_footprint, which counts the
+// plans that a mesh's states share in full for each) fits the HBM budget, beside
+// the plans that finished requests have left idle (which are freed where they
+// stand in the way), and the active-slot limit, gives each admitted request its own non-blocking
 // stream and a resident state, and then keeps every active request's stream
 // fed with `steps_per_launch` large steps at a time, so the work of all
 // active requests overlaps on the device.  Requests that arrive while others
@@ -19,6 +21,7 @@
 #include <condition_variable>
 #include <algorithm>
 #include <deque>
+#include <memory>
 #include <mutex>
 #include <thread>
 #include <unordered_map>
@@ -27,6 +30,9 @@
 #include <cuda_runtime.h>
 
 #include "../../include/sse.h"
+#include "plan_store.h"
+
+std::shared_ptr<sse::PlanStore> sse_internal_plan_store(const sse_mesh *m);   // api.cu
 
 namespace {
 
@@ -79,6 +85,7 @@ struct sse_server {
     int n_active = 0, max_seen_active = 0;
     bool stop = false;
     std::thread worker;
+    std::vector<std::weak_ptr<sse::PlanStore>> stores;   // of the meshes of the requests
     std::vector<cudaStream_t> streams;            // recycled streams and events
     std::vector<cudaEvent_t> events;
 };
@@ -235,6 +242,17 @@ bool packed_round(sse_server *S) {
     return progressed;
 }
 
+// Free the idle plans of the requests' meshes where `bytes` more would not
+// fit the budget beside them (called with S->mu held).
+void make_room(sse_server *S, size_t bytes) {
+    size_t idle = 0;
+    for (auto &w : S->stores)
+        if (auto p = w.lock()) idle += p->idle();
+    if (S->used + bytes + idle <= S->budget) return;
+    for (auto &w : S->stores)
+        if (auto p = w.lock()) p->trim();
+}
+
 void worker_loop(sse_server *S) {
     cudaSetDevice(S->device);
     for (;;) {
@@ -247,6 +265,7 @@ void worker_loop(sse_server *S) {
                    S->n_active + (int)admit.size() < S->max_active) {
                 Req *r = S->pending.front();
                 if (S->used + r->footprint > S->budget) break;
+                make_room(S, r->footprint);
                 S->pending.pop_front();
                 S->used += r->footprint;
                 S->peak = std::max(S->peak, S->used);
@@ -438,6 +457,13 @@ extern "C" int sse_server_submit(sse_server *S, const sse_mesh *mesh, const sse_
         r->id = id;
         r->t_submit = now_s(S->t0);
         try {
+            auto store = sse_internal_plan_store(mesh);
+            auto &known = S->stores;
+            known.erase(std::remove_if(known.begin(), known.end(),
+                                       [](const auto &w) { return w.expired(); }), known.end());
+            if (std::none_of(known.begin(), known.end(),
+                             [&](const auto &w) { return w.lock() == store; }))
+                known.push_back(store);
             S->reqs[id] = r;
             S->pending.push_back(r);
         } catch (...) {

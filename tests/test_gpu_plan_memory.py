@@ -1,5 +1,7 @@
 """Device memory of the patch plans: one copy shared by a mesh's states, found
 again by the states that follow, and nothing left of sse_tune's candidates."""
+import ctypes as ct
+
 import numpy as np
 import pytest
 
@@ -70,3 +72,55 @@ def test_tuning_leaves_no_plans_behind(precision):
     binding.tune_shapes(dm, p, precision, "latency")
     assert binding.plan_bytes(dm) == 0
     dm.close()
+
+
+def _used():
+    """Bytes in use in the device's memory pool, from which states and plans come."""
+    rt = ct.CDLL("libcudart.so.13")
+    pool, out = ct.c_void_p(), ct.c_uint64()
+    assert rt.cudaDeviceSynchronize() == 0
+    assert rt.cudaDeviceGetDefaultMemPool(ct.byref(pool), 0) == 0
+    assert rt.cudaMemPoolGetAttribute(pool, 7, ct.byref(out)) == 0   # cudaMemPoolAttrUsedMemCurrent
+    return out.value
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+@pytest.mark.parametrize("nx,ny", [(16, 32), (48, 60)])
+def test_footprint_covers_the_state_and_its_plans(nx, ny, precision):
+    m, L, p, state = inputs.channel_case(nx, ny, 10e3, 4, perturb=True)
+    dm = binding.Mesh(m, L)
+    fp = binding.footprint(dm, p, precision)
+    assert binding.plan_bytes(dm) == 0
+    before = _used()
+    a = binding.State(dm, p, precision)
+    a.load_state(*state)
+    binding.step_batch([a], 3, [100.0], [6], 1)
+    took = _used() - before
+    # the pool rounds each of about 120 arrays up to 512 bytes, the count to 256
+    assert fp - 120 * 512 <= took <= fp + 120 * 512, (took, fp)
+    a.close()
+    dm.close()
+
+
+def test_idle_plans_stay_inside_a_servers_budget():
+    cases = []
+    for nx, ny in ((48, 60), (40, 66)):
+        m, L, p, state = inputs.channel_case(nx, ny, 10e3, 4, perturb=True)
+        cases.append((binding.Mesh(m, L), p, state))
+
+    def run(budget):
+        srv = binding.Server(hbm_budget=budget, max_active=2)
+        for dm, p, (u, h, tr) in cases:
+            r = srv.submit(dm, p, "mixed", u, h, tr, 3, 100.0, 6, 2)
+            assert r.wait(120)["status"] == "done"
+        srv.close()
+        return [binding.plan_bytes(dm) for dm, _, _ in cases]
+
+    ample = run(1 << 30)
+    assert ample[0] > 0 and ample[1] > 0                # found again by the next request
+    budget = max(binding.footprint(dm, p, "mixed") for dm, p, _ in cases) + min(ample) // 2
+    left = run(budget)
+    # the first mesh's idle plans gave way to the second request
+    assert left[0] == 0 and left[1] > 0
+    for dm, _, _ in cases:
+        dm.close()
