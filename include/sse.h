@@ -240,7 +240,9 @@ int sse_step(sse_state *state, int order, double dt, int n_substeps, int n_steps
  * and thickness kernels (full columns, Algorithm 1, no biharmonic viscosity)
  * with profiling and test hooks off; otherwise SSE_ERR_UNSUPPORTED and no
  * state is stepped.  INVALID_ARG as for sse_step, for n < 1 or for a state
- * listed twice.  Asynchronous. */
+ * listed twice.  Asynchronous, but for a state's first packed call, which may
+ * make and upload its packed launches' plans (a packed request runtime does so
+ * when it admits a request). */
 int sse_step_batch(sse_state *const *states, int n, int order, const double *dt,
                    const int32_t *n_substeps, int n_steps, void *cuda_stream);
 

@@ -33,6 +33,7 @@
 #include "plan_store.h"
 
 std::shared_ptr<sse::PlanStore> sse_internal_plan_store(const sse_mesh *m);   // api.cu
+int sse_internal_prepare_pack(sse_state *st);
 
 namespace {
 
@@ -121,6 +122,7 @@ int start(sse_server *S, Req *r) {
         return SSE_ERR_CUDA;
     }
     int rc = sse_state_create_ex(r->mesh, &r->prm, &r->tun, r->s, &r->st);
+    if (!rc && (S->flags & SSE_SERVER_PACKED)) rc = sse_internal_prepare_pack(r->st);
     if (rc) return rc;
     rc = sse_state_set(r->st, SSE_FIELD_U, r->u.data());
     if (!rc) rc = sse_state_set(r->st, SSE_FIELD_H, r->h.data());
