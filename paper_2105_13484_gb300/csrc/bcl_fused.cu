@@ -114,22 +114,6 @@ template <class R> __device__ __forceinline__ R qdiv(R a, R b);
 template <> __device__ __forceinline__ double qdiv<double>(double a, double b) { return a / b; }
 template <> __device__ __forceinline__ float qdiv<float>(float a, float b) { return __fdividef(a, b); }
 
-// a0 / b0 and a1 / b1.  FP64: one reciprocal of b0 b1 for both (a division is
-// about nine FP64 instructions, and the kernel is bound by that pipe); each
-// quotient is within 2 ulp, in terms (vertical shear and viscosity, potential
-// vorticity) whose error against the exact scheme does not move by it.  Level-7
-// sphere: 15.0 -> 13.8 ms per step.
-__device__ __forceinline__ void div2(float a0, float b0, float a1, float b1, float &q0, float &q1) {
-    q0 = qdiv(a0, b0);
-    q1 = qdiv(a1, b1);
-}
-__device__ __forceinline__ void div2(double a0, double b0, double a1, double b1, double &q0,
-                                     double &q1) {
-    const double r = __drcp_rn(b0 * b1);
-    q0 = a0 * (b1 * r);
-    q1 = a1 * (b0 * r);
-}
-
 // elements of R in n rounded up to 16 bytes
 template <class R> __host__ __device__ __forceinline__ int pad16(int n) {
     return (int)(((size_t)n * sizeof(R) + 15) / 16 * 16 / sizeof(R));
@@ -477,8 +461,8 @@ __device__ __forceinline__ void bcl_fused_patch(const DMesh &m, const DParams &p
             R2 om, qv;
             om.x = bf.x + ot.x;
             om.y = bf.x + ot.y;
-            // (an absent second layer must not spoil the first)
-            div2(bf.y + ot.x, hv.x, bf.y + ot.y, has1 ? hv.y : R(1), qv.x, qv.y);
+            qv.x = qdiv(bf.y + ot.x, hv.x);
+            qv.y = qdiv(bf.y + ot.y, hv.y);
             om_s[v] = om;
             q_s[v] = qv;
         }
@@ -633,14 +617,8 @@ __device__ __forceinline__ void bcl_fused_patch(const DMesh &m, const DParams &p
                     const R u_next = ube + (i ? utn : utc.y);
                     const R he2n = i ? h1n + h2n : h1.y + h2.y;
                     wk1 = i ? W1.y + W2.y : W1.x + W2.x;
-                    if constexpr (sizeof(R) == 8) {
-                        R ih;
-                        div2(u_cur - u_next, he2 + he2n, R(1), he2, Dk1, ih);
-                        vvisc = R(2) * (Xtop - nu_v4 * Dk1) * ih;
-                    } else {
-                        Dk1 = qdiv(u_cur - u_next, he2 + he2n);
-                        vvisc = qdiv(R(2) * (Xtop - nu_v4 * Dk1), he2);
-                    }
+                    Dk1 = qdiv(u_cur - u_next, he2 + he2n);
+                    vvisc = qdiv(R(2) * (Xtop - nu_v4 * Dk1), he2);
                 } else {
                     R utan = R(0);
                     E0Term10<R> tb;   // read again: the bottom layer only
