@@ -148,7 +148,12 @@ __device__ __forceinline__ void transport_cols_edge(const DMesh &m, const Transp
 //   the exchange through a layer's bottom, phibar w - kappa_v D_zt phi, is the
 //     next layer's through its top;
 //   (h phi)1 enters the combination directly (b h1 phi1 = b (h phi)1), so one
-//     division per tracer remains, and the tracers share its reciprocal.
+//     division per tracer remains, and the tracers share its reciprocal;
+//   in FP32 the tracer is formed as an increment of the old level's (of its own
+//     in stage 1), phi_out = t + b ((h phi)1 - h1 t) / h_out with (h phi)1 - h1 t =
+//     h (phi - t) + (h - h1) t + dt (...), so that only increments are rounded:
+//     h phi rounds an absolute tracer (partial bottom cells hold no anomalies) and
+//     its weight at each stage.
 // Level-7 sphere (114,689 cells x 60 layers, T and S), three launches: FP64
 // 10.23 -> 5.47 ms, FP32 0.809 -> 0.781 ms per step (the FP32 kernel waits on
 // loads and barriers, not on arithmetic); errors against the FP64 scheme unchanged.
@@ -351,10 +356,10 @@ __device__ __forceinline__ void thick_fused_patch(const DMesh &m, const DParams 
         const R kvd2 = has2 ? mul_r(kv, rcp_r(mul_r(R(0.5), add_r(hc.y, h_b)))) : R(0);
         // the new thickness: FP64 from the column-integrated flux (volume
         // conservation), and in the tendency precision for the tracers
-        R hor[2], rout[2], bh[2];
+        R hor[2], rout[2], bh[2], dh[2];   // bh: FP64 form; dh = h - h1: FP32 form
 #pragma unroll
         for (int r = 0; r < 2; r++) {
-            hor[r] = R(1); rout[r] = R(1); bh[r] = R(0);
+            hor[r] = R(1); rout[r] = R(1); bh[r] = R(0); dh[r] = R(0);
             if (r && !has1) continue;
             const double share = PB ? m.sfc[x + (size_t)r * Cp] : m.sfrac[k0 + r];
             const double h1 = fma_r(-share, dtD, hs_d[r]);
@@ -363,13 +368,14 @@ __device__ __forceinline__ void thick_fused_patch(const DMesh &m, const DParams 
             hsum += ho;
             if constexpr (sizeof(R) == 8) {
                 hor[r] = ho;
+                bh[r] = mul_r(aR, hnr[r]);
             } else {
                 const R h1r = fma_r(-(r ? sk1 : sk0), dtDr, r ? hc.y : hc.x);
                 hor[r] = comb ? fma_r(aR, hnr[r], mul_r(bR, h1r)) : h1r;
                 a.hR_out[x + (size_t)r * Cp] = hor[r];
+                dh[r] = mul_r(r ? sk1 : sk0, dtDr);
             }
             rout[r] = rcp_r(hor[r]);
-            bh[r] = mul_r(aR, hnr[r]);
         }
 #pragma unroll
         for (int tt = 0; tt < 2; tt++) {
@@ -405,9 +411,18 @@ __device__ __forceinline__ void thick_fused_patch(const DMesh &m, const DParams 
                 if (r && !has1) continue;
                 R rate = fma_r(R(-0.5), r ? adv.y : adv.x, r ? add_r(Xb, -Xm) : add_r(Xm, -Xt));
                 if (KH) rate = add_r(rate, r ? dif.y : dif.x);
-                const R hphi = fma_r(dtR, rate, mul_r(r ? hc.y : hc.x, r ? ph.y : ph.x));
-                const R num = comb ? fma_r(bh[r], trn[r][tt], mul_r(bR, hphi)) : hphi;
-                a.tr_out[(size_t)tt * L * Cp + x + (size_t)r * Cp] = quot(num, hor[r], rout[r]);
+                const R hr = r ? hc.y : hc.x, phr = r ? ph.y : ph.x;
+                R out;
+                if constexpr (sizeof(R) == 8) {
+                    const R hphi = fma_r(dtR, rate, mul_r(hr, phr));
+                    const R num = comb ? fma_r(bh[r], trn[r][tt], mul_r(bR, hphi)) : hphi;
+                    out = quot(num, hor[r], rout[r]);
+                } else {
+                    const R t0 = comb ? trn[r][tt] : phr;
+                    const R inc = fma_r(dtR, rate, fma_r(hr, add_r(phr, -t0), mul_r(dh[r], t0)));
+                    out = add_r(t0, quot(comb ? mul_r(bR, inc) : inc, hor[r], rout[r]));
+                }
+                a.tr_out[(size_t)tt * L * Cp + x + (size_t)r * Cp] = out;
             }
         }
         wk = w2;
