@@ -149,11 +149,6 @@ __device__ __forceinline__ void transport_cols_edge(const DMesh &m, const Transp
 //     next layer's through its top;
 //   (h phi)1 enters the combination directly (b h1 phi1 = b (h phi)1), so one
 //     division per tracer remains, and the tracers share its reciprocal;
-//   in FP32 the tracer is formed as an increment of the old level's (of its own
-//     in stage 1), phi_out = t + b ((h phi)1 - h1 t) / h_out with (h phi)1 - h1 t =
-//     h (phi - t) + (h - h1) t + dt (...), so that only increments are rounded:
-//     h phi rounds an absolute tracer (partial bottom cells hold no anomalies) and
-//     its weight at each stage.
 // Level-7 sphere (114,689 cells x 60 layers, T and S), three launches: FP64
 // 10.23 -> 5.47 ms, FP32 0.809 -> 0.781 ms per step (the FP32 kernel waits on
 // loads and barriers, not on arithmetic); errors against the FP64 scheme unchanged.
@@ -169,7 +164,16 @@ __device__ __forceinline__ void transport_cols_edge(const DMesh &m, const Transp
 // shares are its own, and an edge carries no flux below the layers both its
 // cells have; nothing is written below the column's bottom.  (In place of the
 // unfused kernels, level 6 x 60 layers, mixed: transport and thickness 1.27 ->
-// 0.45 ms per step.)
+// 0.45 ms per step.)  Such meshes hold absolute tracers, which h phi and its
+// Runge-Kutta weights round three times a stage; in FP32 (INC) the tracer is an
+// increment of the old level's t (of its own in stage 1),
+//   phi_out = t + b ((h phi)1 - h1 t) / h_out,
+//   (h phi)1 - h1 t = h (phi - t) + (h - h1) t + dt (...),
+// which rounds it once: the errors of a step against 64 bits go from u 1.9e-6, T
+// 7.3e-8, S 8.0e-8 to 6.1e-7, 4.1e-8, 4.7e-8 in the same time.  Full columns keep
+// h phi: their anomalies are small, and a tracer divided by the rounded h_out
+// compensates its error in rho' h, where the increments' does not (u on 512 cells
+// 3.3e-7 against 3.5e-7).
 template <class R, bool KH, bool PB>
 __device__ __forceinline__ void thick_fused_patch(const DMesh &m, const DParams &p, const DThick &t,
                                                   const ThickFArgs<R> &a, const int pid) {
@@ -184,6 +188,7 @@ __device__ __forceinline__ void thick_fused_patch(const DMesh &m, const DParams 
     const int NP = (L + 1) / 2;   // layer pairs (the second layer of the last is absent if L is odd)
     const int nT = p.nT;
     const bool twoB = a.utB != nullptr, comb = a.a != 0.0;
+    constexpr bool INC = PB && sizeof(R) == 4;
     const PhysR<R> &q = phys<R>(p);
 
     extern __shared__ __align__(16) char smem[];
@@ -356,7 +361,7 @@ __device__ __forceinline__ void thick_fused_patch(const DMesh &m, const DParams 
         const R kvd2 = has2 ? mul_r(kv, rcp_r(mul_r(R(0.5), add_r(hc.y, h_b)))) : R(0);
         // the new thickness: FP64 from the column-integrated flux (volume
         // conservation), and in the tendency precision for the tracers
-        R hor[2], rout[2], bh[2], dh[2];   // bh: FP64 form; dh = h - h1: FP32 form
+        R hor[2], rout[2], bh[2], dh[2];   // bh = a h^n; dh = h - h1 (increments)
 #pragma unroll
         for (int r = 0; r < 2; r++) {
             hor[r] = R(1); rout[r] = R(1); bh[r] = R(0); dh[r] = R(0);
@@ -368,7 +373,6 @@ __device__ __forceinline__ void thick_fused_patch(const DMesh &m, const DParams 
             hsum += ho;
             if constexpr (sizeof(R) == 8) {
                 hor[r] = ho;
-                bh[r] = mul_r(aR, hnr[r]);
             } else {
                 const R h1r = fma_r(-(r ? sk1 : sk0), dtDr, r ? hc.y : hc.x);
                 hor[r] = comb ? fma_r(aR, hnr[r], mul_r(bR, h1r)) : h1r;
@@ -376,6 +380,7 @@ __device__ __forceinline__ void thick_fused_patch(const DMesh &m, const DParams 
                 dh[r] = mul_r(r ? sk1 : sk0, dtDr);
             }
             rout[r] = rcp_r(hor[r]);
+            if (!INC) bh[r] = mul_r(aR, hnr[r]);
         }
 #pragma unroll
         for (int tt = 0; tt < 2; tt++) {
@@ -413,7 +418,7 @@ __device__ __forceinline__ void thick_fused_patch(const DMesh &m, const DParams 
                 if (KH) rate = add_r(rate, r ? dif.y : dif.x);
                 const R hr = r ? hc.y : hc.x, phr = r ? ph.y : ph.x;
                 R out;
-                if constexpr (sizeof(R) == 8) {
+                if constexpr (!INC) {
                     const R hphi = fma_r(dtR, rate, mul_r(hr, phr));
                     const R num = comb ? fma_r(bh[r], trn[r][tt], mul_r(bR, hphi)) : hphi;
                     out = quot(num, hor[r], rout[r]);
