@@ -38,3 +38,27 @@ def test_subcycle_patch_size_keeps_the_bits(name, kw, sizes, order, precision):
     for o in outs[1:]:
         for a, b in zip(o, outs[0]):
             assert np.array_equal(a, b)
+
+
+def test_fp64_without_tensor_memory_takes_the_global_subcycle(monkeypatch):
+    """SSE_BTR_TMEM=0 on the 92,480-cell channel, whose FP64 patches fit an SM
+    only with their edge data in tensor memory: the global-memory sub-cycle
+    runs, within the FP64 parity bound of the oracle."""
+    import oracle
+    m, L, p, (u, h, tr), run = inputs.workload("channel_1km", perturb=True, L=2)
+    o = oracle.Oracle(m, L, p)
+    ubar, _ = o.split(u, h)
+    G = 1e-6 * np.sin(np.arange(m.nEdges) * 0.37)
+    u1, Fz, _ = o.barotropic_substep(3, ubar, o.ssh(h), G, run["dt"], 8)
+    monkeypatch.setenv("SSE_BTR_TMEM", "0")
+    dm = binding.Mesh(m, L)
+    st = binding.State(dm, p, "fp64")
+    assert st.subcycle_shape() == (0, False) and st.patches() == 0
+    st.load_state(u, h, tr)
+    st.set("ubar", ubar)
+    st.set("G", G)
+    st.barotropic_substep(3, run["dt"], 8)
+    for f, ref in (("ubar", u1), ("Fzeta", Fz)):
+        assert np.linalg.norm(st.get(f) - ref) < 1e-11 * np.linalg.norm(ref)
+    st.close()
+    dm.close()
