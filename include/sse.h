@@ -404,9 +404,9 @@ int sse_state_footprint_ex(const sse_mesh *mesh, const sse_params *params,
 
 /* Device bytes of the mesh's patch plans: one copy per plan and precision, made
  * with the first state that needs it and kept for the states that follow.
- * Copies that no state holds are freed with the mesh, behind sse_tune, where
- * device memory runs out while a state is made, and where they stand in the way
- * of a request runtime's budget. */
+ * Copies that no state holds are freed with the mesh, behind sse_tune (those of
+ * the candidates it rejected), where device memory runs out while a state is
+ * made, and where they stand in the way of a request runtime's budget. */
 int sse_mesh_plan_bytes(const sse_mesh *mesh, size_t *bytes);
 
 /* dims = {nCells, nEdges, nVertices, nLayers} of a mesh. */

@@ -5,9 +5,9 @@
 // follow, and kept when the last one goes, so that a state made later on the
 // mesh finds it (on the level-7 sphere a copy costs 42 ms to make, mixed, and
 // a state 8 without).  The idle copies are given back by trim(), which the
-// autotuner calls behind its candidates, the request runtime where they stand in
-// the way of its budget and state creation where memory has run out, and with
-// the store.  Nothing here synchronises the device: a copy is
+// autotuner calls behind its rejected candidates, the request runtime where
+// they stand in the way of its budget and state creation where memory has run
+// out, and with the store.  Nothing here synchronises the device: a copy is
 // complete before any second state can see it, and is freed in stream order
 // behind the work of every state that held it.
 #pragma once
@@ -122,14 +122,15 @@ public:
         leave(it->second, st);
     }
 
-    // Free the copies that no state holds.  Returns their bytes.
-    size_t trim() {
+    // Free the copies that no state holds, but for those in `keep`.  Returns
+    // their bytes.
+    size_t trim(const std::vector<Key> &keep = {}) {
         std::lock_guard<std::mutex> lk(mu_);
         OnDevice dev(device_);
         size_t freed = 0;
         for (auto it = live_.begin(); it != live_.end();) {
             Copy &c = it->second;
-            if (c.holders > 0) {
+            if (c.holders > 0 || std::find(keep.begin(), keep.end(), it->first) != keep.end()) {
                 ++it;
                 continue;
             }
@@ -146,6 +147,12 @@ public:
     }
     ~PlanStore() { trim(); }
 
+    std::vector<Key> keys() {
+        std::lock_guard<std::mutex> lk(mu_);
+        std::vector<Key> out;
+        for (const auto &kv : live_) out.push_back(kv.first);
+        return out;
+    }
     // bytes of all copies, and of those that no state holds
     size_t resident() {
         std::lock_guard<std::mutex> lk(mu_);

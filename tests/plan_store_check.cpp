@@ -127,6 +127,12 @@ int main() {
     S.release(k, st(1));
     S.trim();
     CHECK(allocs.empty() && events.empty());
+    // what is to be kept is kept
+    S.acquire(k, st(1), v, fill); S.release(k, st(1));
+    const auto keep = S.keys();
+    S.acquire(k2, st(1), v, fill); S.release(k2, st(1));
+    CHECK(keep.size() == 1 && S.trim(keep) == 1024 && S.keys() == keep && S.idle() == 1024);
+    CHECK(S.trim() == 1024 && allocs.empty() && events.empty());
     // a store that goes frees what is left
     {
         PlanStore T(0);

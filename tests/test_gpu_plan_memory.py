@@ -1,5 +1,6 @@
 """Device memory of the patch plans: one copy shared by a mesh's states, found
-again by the states that follow, and nothing left of sse_tune's candidates."""
+again by the states that follow, and nothing left of sse_tune's rejected
+candidates."""
 import ctypes as ct
 
 import numpy as np
@@ -59,18 +60,27 @@ def test_a_state_may_outlive_its_mesh_handle():
 
 
 @pytest.mark.parametrize("precision", ["mixed", "fp64"])
-def test_tuning_leaves_no_plans_behind(precision):
-    m, L, p, _ = inputs.channel_case(48, 60, 10e3, 4)
+def test_tuning_leaves_the_chosen_plans_only(precision):
+    m, L, p, state = inputs.channel_case(48, 60, 10e3, 4, perturb=True)
     dm = binding.Mesh(m, L)
-    st = binding.State(dm, p, precision)
-    before = binding.plan_bytes(dm)
-    binding.tune_shapes(dm, p, precision, "throughput")
-    assert binding.plan_bytes(dm) == before
-    st.close()
-    dm.close()
-    dm = binding.Mesh(m, L)
-    binding.tune_shapes(dm, p, precision, "latency")
-    assert binding.plan_bytes(dm) == 0
+    for objective in ("throughput", "latency"):
+        before = binding.plan_bytes(dm)
+        shapes = binding.tune_shapes(dm, p, precision, objective)
+        after = binding.plan_bytes(dm)
+        # a state of these shapes, alone and packed, finds all it needs ...
+        st = binding.State(dm, p, precision, **shapes)
+        st.load_state(*state)
+        binding.step_batch([st], 3, [100.0], [6], 1)
+        assert binding.plan_bytes(dm) == after
+        st.close()
+        # ... and nothing else was left
+        fresh = binding.Mesh(m, L)
+        st = binding.State(fresh, p, precision, **shapes)
+        st.load_state(*state)
+        binding.step_batch([st], 3, [100.0], [6], 1)
+        assert after - before <= binding.plan_bytes(fresh)
+        st.close()
+        fresh.close()
     dm.close()
 
 
