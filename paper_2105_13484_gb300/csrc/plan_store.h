@@ -170,7 +170,8 @@ private:
     struct OnDevice {
         int was = -1;
         explicit OnDevice(int dev) {
-            if (cudaGetDevice(&was) != cudaSuccess || was == dev || cudaSetDevice(dev) != cudaSuccess)
+            if (cudaGetDevice(&was) != cudaSuccess || was == dev ||
+                cudaSetDevice(dev) != cudaSuccess)
                 was = -1;
         }
         ~OnDevice() {
