@@ -134,3 +134,49 @@ def test_idle_plans_stay_inside_a_servers_budget():
     assert left[0] == 0 and left[1] > 0
     for dm, _, _ in cases:
         dm.close()
+
+
+def test_threads_share_plans_while_others_tune_and_go():
+    """States come, step and go on several threads and streams while sse_tune
+    frees idle plans of the same mesh: the bits are those of a state alone."""
+    import threading
+
+    torch = pytest.importorskip("torch")
+    m, L, p, state = inputs.channel_case(48, 60, 10e3, 4, perturb=True)
+    dm = binding.Mesh(m, L)
+    ref = {}
+    for precision in ("mixed", "fp64"):
+        st = binding.State(dm, p, precision)
+        st.load_state(*state)
+        st.step(3, 100.0, 6, 3)
+        ref[precision] = st.read_state()
+        st.close()
+    wrong = []
+
+    def work(k):
+        try:
+            stream = torch.cuda.Stream()
+            for i in range(6):
+                precision = ("mixed", "fp64")[(i + k) % 2]
+                st = binding.State(dm, p, precision, stream=stream.cuda_stream,
+                                   patch_cells=(0, 128)[i % 2])
+                st.load_state(*state)
+                st.step(3, 100.0, 6, 3)
+                got = st.read_state()
+                st.step(3, 100.0, 6, 3)   # goes with work in flight
+                st.close()
+                if not all(np.array_equal(a, b) for a, b in zip(got, ref[precision])):
+                    wrong.append((k, i))
+        except Exception as e:   # noqa: BLE001 - reported by the assertion below
+            wrong.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(4)]
+    for t in threads:
+        t.start()
+    for precision in ("mixed", "fp64"):
+        for objective in ("latency", "throughput"):
+            binding.tune_shapes(dm, p, precision, objective)
+    for t in threads:
+        t.join()
+    assert not wrong, wrong
+    dm.close()
